@@ -163,6 +163,9 @@ perf_status check_options(const perf_options* o, std::string& why) {
     return PERF_OK;
 }
 
+// DevScene::cap_per_sm of a resident grid of as many CTAs as fit.
+constexpr int kResident = 32;
+
 // Objectives in flight: a Gauss-Newton step's F(x) and two trial points; the
 // second is also perf_sample_count's.
 constexpr int kFSlots = 3;
@@ -369,11 +372,40 @@ bool copies_ready(perf_ctx* ctx, CopyNeed what, cudaStream_t st) {
            cudaStreamWaitEvent(st, ctx->copy_ev, 0) == cudaSuccess;
 }
 
+int scatter_spread(const perf_ctx* ctx) {
+    return perf::scatter_spread_of(ctx->ds.n_tiles, ctx->n_rays, ctx->n);
+}
+
+// scatter_spread for the marches of a solve: the diagonal and A p in the spread
+// order and from copies, or in the plain order from x and p on a resident grid,
+// which repeats its order of additions more closely from run to run (of the
+// voxels that a few rays see, twice as many keep their sum to the last bit).
+// What magnifies a last bit asks for that: the inverse of a voxel's block that
+// those rays leave singular (x after a step of the block Jacobi preconditioner
+// moved by up to 7e-2 of its norm where two plain runs differ by 1e-5), and p
+// and x rounded to BF16 (F by up to 4e-4 against 5e-6).  128^3, 12 x 800^2, 10
+// iterations: 151 ms spread, 190 plain.
+int solver_spread(const perf_ctx* ctx) {
+    if (ctx->scene.dtype == PERF_BF16 || ctx->opts.precond == PERF_PRECOND_BLOCK_JACOBI) return 0;
+    return scatter_spread(ctx);
+}
+
+// d for a solve's scatters without copies, resident where the spread order is
+// left for the plain one.
+void plain_scatter(const perf_ctx* ctx, perf::DevScene& d) {
+    d.xcopy = nullptr;
+    d.pcopy = nullptr;
+    d.sigma8 = nullptr;
+    d.spread = solver_spread(ctx);
+    if (ctx->ds.spread && !d.spread && d.cap_per_sm == 0) d.cap_per_sm = kResident;
+}
+
 // d = the context's scene with the gather copies of x (and, with kNeedP, of p
 // in type p_dtype), made on st, where they pay.
 perf_status gather_copies(perf_ctx* ctx, const void* x, const void* p, int p_dtype, CopyNeed what,
                           cudaStream_t st, perf::DevScene& d) {
     d = ctx->ds;
+    if (what != kNeedX) d.spread = scatter_spread(ctx);
     if (!copies_ready(ctx, what, st)) return PERF_OK;
     CK(perf::launch_gather_copy(d.n_vox, d.G, ctx->scene.dtype, x, ctx->xcopy,
                                 what >= kNeedSigma ? ctx->sigma8 : nullptr, st, p_dtype, p, ctx->pcopy));
@@ -823,8 +855,14 @@ perf_status perf_pcg_step(perf_ctx* ctx, const void* x, int32_t* done_out, void*
     SHELLS(ctx, S(stream));
     perf::DevScene d;
     const bool bf = ctx->scene.dtype == PERF_BF16;
-    perf_status st = gather_copies(ctx, x, bf ? static_cast<const void*>(ctx->p16) : ctx->p,
-                                   ctx->scene.dtype, kNeedP, S(stream), d);
+    perf_status st = PERF_OK;
+    if (solver_spread(ctx)) {
+        st = gather_copies(ctx, x, bf ? static_cast<const void*>(ctx->p16) : ctx->p, ctx->scene.dtype,
+                           kNeedP, S(stream), d);
+    } else {
+        d = ctx->ds;
+        plain_scatter(ctx, d);
+    }
     if (st == PERF_OK) st = pcg_iter(ctx, x, ctx->diag, B, S(stream), false, d);
     if (st == PERF_OK) st = copies_done(ctx, d, S(stream));
     if (st != PERF_OK) return st;
@@ -890,16 +928,18 @@ perf_status perf_gn_solve(perf_ctx* ctx, float* x, const void* target, int32_t n
         CK(cudaMemsetAsync(ctx->dF, 0, sizeof(double), st));
         // the step's marches of x read its gather copy, the A p that of p
         perf::DevScene ds = ctx->ds;
-        const bool copies = ctx->n_rays > 0 && copies_ready(ctx, kNeedP, st);
-        if (copies) {
-            ds.xcopy = ctx->xcopy;
+        const int spread = solver_spread(ctx);
+        const bool copies = ctx->n_rays > 0 && copies_ready(ctx, spread ? kNeedP : kNeedX, st);
+        const bool scatter_copies = copies && spread;
+        if (copies) ds.xcopy = ctx->xcopy;
+        if (scatter_copies) {
             ds.sigma8 = ctx->sigma8;
             ds.diag2 = ctx->diag2;
         }
-        const bool scatter_copies = copies && ds.spread;
         t_begin(ctx, PERF_T_RESIDUAL, st);
         if (copies)
-            CK(perf::launch_gather_copy(ds.n_vox, ds.G, ctx->scene.dtype, xm, ctx->xcopy, ctx->sigma8, st));
+            CK(perf::launch_gather_copy(ds.n_vox, ds.G, ctx->scene.dtype, xm, ctx->xcopy,
+                                        scatter_copies ? ctx->sigma8 : nullptr, st));
         if (ctx->n_rays > 0)
             CK(perf::launch_forward(ds, ctx->scene.dtype, xm, target, ctx->r, nullptr, ctx->dF, 1, st));
         t_end(ctx, PERF_T_RESIDUAL, st);
@@ -924,10 +964,8 @@ perf_status perf_gn_solve(perf_ctx* ctx, float* x, const void* target, int32_t n
         // per voxel; the learned network and caller-given blocks read the
         // canonical order
         perf::DevScene dl = ds;
-        if (!scatter_copies) {
-            dl.xcopy = nullptr;
-            dl.sigma8 = nullptr;
-        }
+        dl.spread = spread;
+        if (!scatter_copies) plain_scatter(ctx, dl);
         perf::set_layout(dl, (use_coef && ctx->coef_tiles >= ctx->ds.n_tiles &&
                               o.precond != PERF_PRECOND_BLOCK4) ? ctx->brick_s : 0);
         dl.keff = use_coef ? ctx->keff : nullptr;
@@ -1149,6 +1187,8 @@ static perf_status autotune_impl(perf_ctx* ctx, const void* x, const void* p, pe
         d.pcopy = dc.pcopy;
         d.sigma8 = dc.sigma8;
         d.diag2 = dc.diag2;
+        d.spread = solver_spread(ctx);
+        if (!d.spread) plain_scatter(ctx, d);
         return d;
     };
     const int tws[4] = {8, 4, 16, 32};

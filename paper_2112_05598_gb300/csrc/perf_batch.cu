@@ -130,7 +130,8 @@ perf_status apply_tiling(perf_batch* b, int tw) {
     }
     start[b->n] = t;
     b->total_tiles = t;
-    for (BatchItem& it : b->items) it.sc.spread = perf::spread_of(t);
+    for (int i = 0; i < b->n; ++i)
+        b->items[i].sc.spread = perf::scatter_spread_of(t, b->items[i].sc.n_rays, 4 * (b->seg_h[i + 1] - b->seg_h[i]));
     BK(cudaMemcpy(b->d_items, b->items.data(), sizeof(BatchItem) * b->n, cudaMemcpyHostToDevice));
     BK(cudaMemcpy(b->d_start, start.data(), sizeof(long long) * (b->n + 1), cudaMemcpyHostToDevice));
     if (b->graph) {

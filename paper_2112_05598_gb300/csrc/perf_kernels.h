@@ -87,6 +87,19 @@ struct PcgScalars {
 // 1889, 6565 / 5072.
 inline int spread_of(long long tiles) { return tiles >= 152 * 10 ? 3 : 0; }
 
+// The same for a march that scatters.  A parameter that very many rays see is a
+// long chain of binary32 additions, and what it rounds to follows the order of
+// the chain, run after run.  Either order is as exact (A p at 2^3, 92 k rays:
+// 5.8 to 7.9e-6 off plain, 6.9 to 8.5e-6 spread), but a Gauss-Newton step of a
+// small system turns the difference into its objective, so scenes with more
+// than 32 residuals a parameter keep the plain order, the one that small
+// launches have too.  F after a step, relative difference of the two orders (of
+// two runs of one: 1e-6): 1 to 8e-5 at 25^3 to 36^3 with 50 to 110 residuals a
+// parameter, at most 6e-6 up to 32 (1e-7 at 128^3, 100 x 800^2: 19).
+inline int scatter_spread_of(long long tiles, long long rays, long long params) {
+    return 3 * rays > 32 * params ? 0 : spread_of(tiles);
+}
+
 // Sets the parameter-vector block order of d (see LayoutKey): s = 0 the
 // canonical order, s > 0 bricks of 2^s voxels per edge.  Returns false (and
 // leaves d canonical) when G is not a multiple of the brick edge.
