@@ -77,8 +77,8 @@ struct perf_ctx {
     bool coef_used = false;            // the last Gauss-Newton step used the store
     float* Ap = nullptr;
     // gather copies of the march in hand (see GatherKey in perf_device.cuh): of
-    // x, of the vector J acts on, and x's opacity records.  A call on another
-    // stream than the last waits for copy_ev, recorded behind every use.
+    // x, of the vector J acts on, and x's opacity records.  Every use waits for
+    // copy_ev, recorded behind the last one (CopyUse).
     // One allocation, as large as any call has needed.
     void* copies = nullptr;
     size_t copies_bytes = 0;
@@ -86,7 +86,6 @@ struct perf_ctx {
     float* sigma8 = nullptr;
     float2* diag2 = nullptr;    // packed sums of the diagonal march, n / 4 blocks
     cudaEvent_t copy_ev = nullptr;
-    cudaStream_t copy_st = nullptr;
     bool copy_used = false;
     // shell hits of every ray (n_rays x S entries, FP64 texel coordinates),
     // valid for jitter epoch shell_tab_epoch (-1: no jitter); see ensure_shells
@@ -336,11 +335,39 @@ bool copies_pay(const perf_ctx* ctx, CopyNeed what) {
            samples >= perf::kCopyRatio * (double)ctx->ds.n_vox;
 }
 
-// Room for the gather copies of a march on st, free of earlier calls' use;
+// A call's use of the gather copies on st: from take() on, whatever way the
+// call is left, the event that the next use waits for is recorded behind what
+// the call has queued.
+struct CopyUse {
+    perf_ctx* ctx;
+    cudaStream_t st;
+    bool on = false;
+    CopyUse(perf_ctx* c, cudaStream_t s) : ctx(c), st(s) {}
+    CopyUse(const CopyUse&) = delete;
+    CopyUse& operator=(const CopyUse&) = delete;
+    // Waits for the last use, on whichever stream it was: equal handles need not
+    // be one stream (a host thread's default stream, a handle used again).
+    bool take() {
+        if (ctx->copy_used && cudaStreamWaitEvent(st, ctx->copy_ev, 0) != cudaSuccess) {
+            cudaGetLastError();
+            return false;
+        }
+        on = true;
+        return true;
+    }
+    ~CopyUse() {
+        if (!on) return;
+        ctx->copy_used = true;
+        if (cudaEventRecord(ctx->copy_ev, st) != cudaSuccess) cudaStreamSynchronize(st);
+    }
+};
+
+// Room for the gather copies of a march on use.st, free of earlier calls' use;
 // false: the march gathers from x and p themselves -- few samples, no memory,
 // or a stream under capture, whose graph would keep the workspace.
-bool copies_ready(perf_ctx* ctx, CopyNeed what, cudaStream_t st) {
+bool copies_ready(perf_ctx* ctx, CopyNeed what, CopyUse& use) {
     if (!copies_pay(ctx, what)) return false;
+    const cudaStream_t st = use.st;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
         cudaGetLastError();
@@ -366,10 +393,11 @@ bool copies_ready(perf_ctx* ctx, CopyNeed what, cudaStream_t st) {
         ctx->diag2 = reinterpret_cast<float2*>(ctx->sigma8 + 8 * nv);
         ctx->pcopy = reinterpret_cast<float4*>(ctx->diag2 + nb);
     }
-    if (!ctx->copy_ev && cudaEventCreateWithFlags(&ctx->copy_ev, cudaEventDisableTiming) != cudaSuccess)
+    if (!ctx->copy_ev && cudaEventCreateWithFlags(&ctx->copy_ev, cudaEventDisableTiming) != cudaSuccess) {
+        cudaGetLastError();
         return false;
-    return !(ctx->copy_used && ctx->copy_st != st) ||
-           cudaStreamWaitEvent(st, ctx->copy_ev, 0) == cudaSuccess;
+    }
+    return use.take();
 }
 
 int scatter_spread(const perf_ctx* ctx) {
@@ -401,14 +429,15 @@ void plain_scatter(const perf_ctx* ctx, perf::DevScene& d) {
 }
 
 // d = the context's scene with the gather copies of x (and, with kNeedP, of p
-// in type p_dtype), made on st, where they pay.
+// in type p_dtype), made on use.st, where they pay.
 perf_status gather_copies(perf_ctx* ctx, const void* x, const void* p, int p_dtype, CopyNeed what,
-                          cudaStream_t st, perf::DevScene& d) {
+                          CopyUse& use, perf::DevScene& d) {
     d = ctx->ds;
     if (what != kNeedX) d.spread = scatter_spread(ctx);
-    if (!copies_ready(ctx, what, st)) return PERF_OK;
+    if (!copies_ready(ctx, what, use)) return PERF_OK;
     CK(perf::launch_gather_copy(d.n_vox, d.G, ctx->scene.dtype, x, ctx->xcopy,
-                                what >= kNeedSigma ? ctx->sigma8 : nullptr, st, p_dtype, p, ctx->pcopy));
+                                what >= kNeedSigma ? ctx->sigma8 : nullptr, use.st, p_dtype, p,
+                                ctx->pcopy));
     d.xcopy = ctx->xcopy;
     d.pcopy = p ? ctx->pcopy : nullptr;
     d.sigma8 = ctx->sigma8;
@@ -429,19 +458,12 @@ perf_status diag_march(perf_ctx* ctx, const perf::DevScene& d, const void* x, co
     return PERF_OK;
 }
 
-perf_status copies_done(perf_ctx* ctx, const perf::DevScene& d, cudaStream_t st) {
-    if (!d.xcopy) return PERF_OK;
-    CK(cudaEventRecord(ctx->copy_ev, st));
-    ctx->copy_st = st;
-    ctx->copy_used = true;
-    return PERF_OK;
-}
-
-#define COPIES(ctx, x, p, what, st, d)                                           \
-    perf::DevScene d;                                                            \
-    do {                                                                         \
-        const perf_status ps_ = gather_copies(ctx, x, p, PERF_F32, what, st, d); \
-        if (ps_ != PERF_OK) return ps_;                                          \
+#define COPIES(ctx, x, p, what, st, d)                                            \
+    perf::DevScene d;                                                             \
+    CopyUse use_(ctx, st);                                                        \
+    do {                                                                          \
+        const perf_status ps_ = gather_copies(ctx, x, p, PERF_F32, what, use_, d); \
+        if (ps_ != PERF_OK) return ps_;                                           \
     } while (0)
 
 void t_begin(perf_ctx* c, int k, cudaStream_t st) {
@@ -646,7 +668,7 @@ perf_status perf_render(perf_ctx* ctx, const void* x, float* rgb_out, float* T_o
     SHELLS(ctx, S(stream));
     COPIES(ctx, x, nullptr, kNeedX, S(stream), d);
     CK(perf::launch_forward(d, ctx->scene.dtype, x, nullptr, rgb_out, T_out, nullptr, 0, S(stream)));
-    return copies_done(ctx, d, S(stream));
+    return PERF_OK;
 }
 
 perf_status perf_residual(perf_ctx* ctx, const void* x, const void* target, void* r_out,
@@ -660,7 +682,7 @@ perf_status perf_residual(perf_ctx* ctx, const void* x, const void* target, void
     COPIES(ctx, x, nullptr, kNeedX, S(stream), d);
     CK(perf::launch_forward(d, ctx->scene.dtype, x, target, r_out, nullptr, F_out,
                             r_out ? 1 : 2, S(stream)));
-    return copies_done(ctx, d, S(stream));
+    return PERF_OK;
 }
 
 perf_status perf_jvp(perf_ctx* ctx, const void* x, const float* p, float* jp_out, void* stream) {
@@ -670,7 +692,7 @@ perf_status perf_jvp(perf_ctx* ctx, const void* x, const float* p, float* jp_out
     SHELLS(ctx, S(stream));
     COPIES(ctx, x, p, kNeedP, S(stream), d);
     CK(perf::launch_jvp(d, ctx->scene.dtype, x, p, PERF_F32, jp_out, S(stream)));
-    return copies_done(ctx, d, S(stream));
+    return PERF_OK;
 }
 
 perf_status perf_vjp(perf_ctx* ctx, const void* x, const float* v, float* out, int32_t accumulate,
@@ -684,7 +706,7 @@ perf_status perf_vjp(perf_ctx* ctx, const void* x, const float* v, float* out, i
     COPIES(ctx, x, nullptr, kNeedSigma, S(stream), d);
     CK(perf::launch_scatter(d, ctx->scene.dtype, 0, x, nullptr, PERF_F32, v, out, nullptr,
                             nullptr, S(stream)));
-    return copies_done(ctx, d, S(stream));
+    return PERF_OK;
 }
 
 perf_status perf_diag_jtj(perf_ctx* ctx, const void* x, const void* r, float* diag_out,
@@ -702,7 +724,7 @@ perf_status perf_diag_jtj(perf_ctx* ctx, const void* x, const void* r, float* di
     SHELLS(ctx, S(stream));
     COPIES(ctx, x, nullptr, kNeedDiag, S(stream), d);
     const perf_status ps = diag_march(ctx, d, x, r, diag_out, grad_out, nullptr, nullptr, nullptr, S(stream));
-    return ps != PERF_OK ? ps : copies_done(ctx, d, S(stream));
+    return ps;
 }
 
 perf_status perf_apply_normal(perf_ctx* ctx, const void* x, const float* p, float* ap_out,
@@ -717,7 +739,7 @@ perf_status perf_apply_normal(perf_ctx* ctx, const void* x, const float* p, floa
     COPIES(ctx, x, p, kNeedP, S(stream), d);
     CK(perf::launch_scatter(d, ctx->scene.dtype, 1, x, p, PERF_F32, nullptr, ap_out, nullptr,
                             pap_out, S(stream)));
-    return copies_done(ctx, d, S(stream));
+    return PERF_OK;
 }
 
 perf_status perf_pcg_begin(perf_ctx* ctx, const float* grad, const float* diag, void* stream) {
@@ -856,15 +878,15 @@ perf_status perf_pcg_step(perf_ctx* ctx, const void* x, int32_t* done_out, void*
     perf::DevScene d;
     const bool bf = ctx->scene.dtype == PERF_BF16;
     perf_status st = PERF_OK;
+    CopyUse use(ctx, S(stream));
     if (solver_spread(ctx)) {
         st = gather_copies(ctx, x, bf ? static_cast<const void*>(ctx->p16) : ctx->p, ctx->scene.dtype,
-                           kNeedP, S(stream), d);
+                           kNeedP, use, d);
     } else {
         d = ctx->ds;
         plain_scatter(ctx, d);
     }
     if (st == PERF_OK) st = pcg_iter(ctx, x, ctx->diag, B, S(stream), false, d);
-    if (st == PERF_OK) st = copies_done(ctx, d, S(stream));
     if (st != PERF_OK) return st;
     if (done_out) {
         int done = 0;
@@ -915,6 +937,7 @@ perf_status perf_gn_solve(perf_ctx* ctx, float* x, const void* target, int32_t n
     const perf_options& o = ctx->opts;
     const uint32_t epoch0 = o.epoch;
     perf_status result = PERF_OK;
+    CopyUse use(ctx, st);
     for (int step = 0; step < n_steps; ++step) {
         ctx->ds.epoch = epoch0 + (uint32_t)step;
         SHELLS(ctx, st);
@@ -929,7 +952,7 @@ perf_status perf_gn_solve(perf_ctx* ctx, float* x, const void* target, int32_t n
         // the step's marches of x read its gather copy, the A p that of p
         perf::DevScene ds = ctx->ds;
         const int spread = solver_spread(ctx);
-        const bool copies = ctx->n_rays > 0 && copies_ready(ctx, spread ? kNeedP : kNeedX, st);
+        const bool copies = ctx->n_rays > 0 && copies_ready(ctx, spread ? kNeedP : kNeedX, use);
         const bool scatter_copies = copies && spread;
         if (copies) ds.xcopy = ctx->xcopy;
         if (scatter_copies) {
@@ -1140,11 +1163,6 @@ perf_status perf_gn_solve(perf_ctx* ctx, float* x, const void* target, int32_t n
         if (result != PERF_OK) break;
     }
     ctx->ds.epoch = epoch0;
-    if (ctx->copy_ev) {   // the stream is idle: the next call on any stream may use the copies
-        CK(cudaEventRecord(ctx->copy_ev, st));
-        ctx->copy_st = st;
-        ctx->copy_used = true;
-    }
     if (result == PERF_ERR_NONFINITE) return fail(ctx, result, "gn_solve: non-finite objective");
     return result;
 }
@@ -1179,7 +1197,8 @@ static perf_status autotune_impl(perf_ctx* ctx, const void* x, const void* p, pe
     const void* pp = pbuf;
     // the solver's A p gathers from copies where they pay: so does the tuner's
     perf::DevScene dc;
-    ps = gather_copies(ctx, x, pp, ctx->scene.dtype, kNeedP, st, dc);
+    CopyUse use(ctx, st);
+    ps = gather_copies(ctx, x, pp, ctx->scene.dtype, kNeedP, use, dc);
     if (ps != PERF_OK) return ps;
     auto scene = [&]() {
         perf::DevScene d = ctx->ds;
@@ -1370,7 +1389,7 @@ perf_status perf_diag_cross(perf_ctx* ctx, const void* x, float* diag_out, float
     SHELLS(ctx, S(stream));
     COPIES(ctx, x, nullptr, kNeedDiag, S(stream), d);
     const perf_status ps = diag_march(ctx, d, x, nullptr, diag_out, nullptr, cross_out, nullptr, nullptr, S(stream));
-    return ps != PERF_OK ? ps : copies_done(ctx, d, S(stream));
+    return ps;
 }
 
 perf_status perf_adam_step(perf_ctx* ctx, float* x, const void* target, float* m, float* v,
@@ -1397,8 +1416,6 @@ perf_status perf_adam_step(perf_ctx* ctx, float* x, const void* target, float* m
         CK(perf::launch_forward(d, PERF_F32, x, target, ctx->r, nullptr, ctx->dF, 1, st));
         CK(perf::launch_scatter(d, PERF_F32, 0, x, nullptr, PERF_F32, ctx->r, ctx->grad, nullptr,
                                 nullptr, st));
-        ps = copies_done(ctx, d, st);
-        if (ps != PERF_OK) return ps;
     }
     const float c1 = 1.0f - std::pow(beta1, (float)t), c2 = 1.0f - std::pow(beta2, (float)t);
     CK(perf::launch_adam(ctx->n, x, ctx->grad, m, v, beta1, beta2, lr, eps, c1, c2,
@@ -1500,7 +1517,7 @@ perf_status perf_render_threshold(perf_ctx* ctx, const void* x, float min_opacit
     COPIES(ctx, x, nullptr, kNeedX, S(stream), d);
     CK(perf::launch_forward(d, ctx->scene.dtype, x, nullptr, rgb_out, T_out, nullptr, 0, S(stream),
                             min_opacity));
-    return copies_done(ctx, d, S(stream));
+    return PERF_OK;
 }
 
 perf_status perf_upsample(const float* x, int32_t G, int32_t n_shells, int32_t env_h,
