@@ -379,6 +379,7 @@ bool copies_ready(perf_ctx* ctx, CopyNeed what, CopyUse& use) {
     if (what >= kNeedSigma) need += 8 * sizeof(float) * nv;
     if (what >= kNeedDiag) need += sizeof(float2) * nb;
     if (what >= kNeedP) need += sizeof(float4) * ng;
+    const perf::BesideCapture beside;
     if (ctx->copies_bytes < need) {
         if (ctx->copies) cudaFree(ctx->copies);   // (waits for its users)
         ctx->copies = nullptr;

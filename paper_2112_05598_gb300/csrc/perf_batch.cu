@@ -159,6 +159,7 @@ bool copies_ready(perf_batch* b, cudaStream_t st) {
         cudaGetLastError();
         return false;
     }
+    const perf::BesideCapture beside;
     size_t ng = 0, nv = 0;
     for (const BatchItem& it : b->items) {
         ng += (size_t)perf::gather_size(it.sc.G);

@@ -162,6 +162,17 @@ struct GatherDst {
     int bf16;              // 1: the gathered p is BF16 (the copy holds its rounded values)
 };
 
+// While it lives, this thread's allocations are allowed beside a capture on
+// another stream (which they would otherwise end): a march that is not captured
+// may make its workspace at any time.
+struct BesideCapture {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    BesideCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+    ~BesideCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+    BesideCapture(const BesideCapture&) = delete;
+    BesideCapture& operator=(const BesideCapture&) = delete;
+};
+
 // Total grid samples and shell hits over all rays (one march of the scene).
 cudaError_t launch_count_samples(const DevScene& sc, unsigned long long* out, cudaStream_t st);
 

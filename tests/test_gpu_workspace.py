@@ -96,3 +96,31 @@ def test_a_call_after_a_failed_solve_waits_for_its_marches():
         ctx.render(xs[1], out, stream=b)
         torch.cuda.synchronize()
         assert torch.equal(out, want[1])
+
+
+def test_first_calls_leave_a_capture_on_another_stream_alone():
+    """Calls on a stream that is not under capture may allocate their workspace
+    while another stream of the thread is: the capture goes on."""
+    import torch
+    from paper_2112_05598_gb300 import Batch
+    from scenegen import make_cameras, random_params
+    ctx, xs = _context(G=32, W=300, cams=4)
+    want = _reference(*_context(G=32, W=300, cams=4))[0]
+    rng = np.random.default_rng(3)
+    c2w, focal = make_cameras(rng, 4, 200, 3.2, "sphere", 40.0)
+    batch = Batch([dict(G=24, radii=(), env_h=0, env_w=0, c2w=c2w, focal=focal, width=200, height=200)] * 2)
+    xb = cuda_tensor(np.concatenate([random_params(rng, 24, 0, 0, 0, 0.01, 0.2)] * 2))
+    out, diag, rgb, y = empty(3 * ctx.n_rays), empty(xs[0].numel()), empty(3 * batch.n_rays), empty(4)
+    other, graph = torch.cuda.Stream(), torch.cuda.CUDAGraph()
+    torch.cuda.synchronize()
+    with torch.cuda.graph(graph):
+        y.add_(1.0)
+        ctx.render(xs[0], out, stream=other)
+        ctx.diag_jtj(xs[0], diag, stream=other)
+        batch.render(xb, rgb, stream=other)
+        y.add_(1.0)
+    torch.cuda.synchronize()
+    assert torch.equal(out, want) and float(diag.sum()) > 0 and float(rgb.sum()) > 0
+    graph.replay()
+    torch.cuda.synchronize()
+    assert y.tolist() == [2.0] * 4
