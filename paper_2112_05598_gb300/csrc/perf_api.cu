@@ -79,9 +79,10 @@ struct perf_ctx {
     // gather copies of the march in hand (see GatherKey in perf_device.cuh): of
     // x, of the vector J acts on, and x's opacity records.  Every use waits for
     // copy_ev, recorded behind the last one (CopyUse).
-    // One allocation, as large as any call has needed.
-    void* copies = nullptr;
-    size_t copies_bytes = 0;
+    // Allocated as calls need them (CopyNeed), a call's missing parts together,
+    // and kept: growing frees nothing, which would wait for the marches in flight.
+    void* copies[4] = {nullptr, nullptr, nullptr, nullptr};
+    int copies_made = 0;        // parts, in CopyNeed's order
     float4 *xcopy = nullptr, *pcopy = nullptr;
     float* sigma8 = nullptr;
     float2* diag2 = nullptr;    // packed sums of the diagonal march, n / 4 blocks
@@ -373,26 +374,30 @@ bool copies_ready(perf_ctx* ctx, CopyNeed what, CopyUse& use) {
         cudaGetLastError();
         return false;
     }
-    const size_t ng = (size_t)perf::gather_size(ctx->ds.G), nv = (size_t)ctx->ds.n_vox,
-                 nb = ((size_t)ctx->n / 4 + 1) / 2 * 2;
-    size_t need = sizeof(float4) * ng;
-    if (what >= kNeedSigma) need += 8 * sizeof(float) * nv;
-    if (what >= kNeedDiag) need += sizeof(float2) * nb;
-    if (what >= kNeedP) need += sizeof(float4) * ng;
     const perf::BesideCapture beside;
-    if (ctx->copies_bytes < need) {
-        if (ctx->copies) cudaFree(ctx->copies);   // (waits for its users)
-        ctx->copies = nullptr;
-        ctx->copies_bytes = 0;
-        if (cudaMalloc(&ctx->copies, need) != cudaSuccess) {
+    if (ctx->copies_made <= what) {
+        // the parts that earlier calls did not need, in one allocation
+        const size_t ng = sizeof(float4) * (size_t)perf::gather_size(ctx->ds.G);
+        const size_t bytes[4] = {ng, 8 * sizeof(float) * (size_t)ctx->ds.n_vox,
+                                 sizeof(float2) * (((size_t)ctx->n / 4 + 1) / 2 * 2), ng};
+        size_t need = 0;
+        for (int q = ctx->copies_made; q <= what; ++q) need += bytes[q];
+        char* at = nullptr;
+        if (cudaMalloc(&at, need) != cudaSuccess) {
             cudaGetLastError();
             return false;
         }
-        ctx->copies_bytes = need;
-        ctx->xcopy = static_cast<float4*>(ctx->copies);
-        ctx->sigma8 = reinterpret_cast<float*>(ctx->xcopy + ng);
-        ctx->diag2 = reinterpret_cast<float2*>(ctx->sigma8 + 8 * nv);
-        ctx->pcopy = reinterpret_cast<float4*>(ctx->diag2 + nb);
+        ctx->copies[ctx->copies_made] = at;
+        for (; ctx->copies_made <= what; ++ctx->copies_made) {
+            void* part = at;
+            switch (ctx->copies_made) {
+                case kNeedX: ctx->xcopy = static_cast<float4*>(part); break;
+                case kNeedSigma: ctx->sigma8 = static_cast<float*>(part); break;
+                case kNeedDiag: ctx->diag2 = static_cast<float2*>(part); break;
+                default: ctx->pcopy = static_cast<float4*>(part);
+            }
+            at += bytes[ctx->copies_made];
+        }
     }
     if (!ctx->copy_ev && cudaEventCreateWithFlags(&ctx->copy_ev, cudaEventDisableTiming) != cudaSuccess) {
         cudaGetLastError();
@@ -621,7 +626,7 @@ perf_status perf_create(perf_ctx** out, const perf_scene* sc, const perf_cameras
 perf_status perf_destroy(perf_ctx* ctx) {
     if (!ctx) return PERF_ERR_INVALID_ARG;
     void* bufs[] = {ctx->cams, ctx->r, ctx->diag, ctx->grad, ctx->delta, ctx->rho, ctx->p,
-                    ctx->Ap, ctx->copies, ctx->tile_off, ctx->coef, ctx->keff, ctx->d_prefix, ctx->shell_tab, ctx->hist, ctx->cross, ctx->blocks_ws, ctx->feat, ctx->x_trial, ctx->x16, ctx->p16, ctx->t16, ctx->s, ctx->dF};
+                    ctx->Ap, ctx->copies[0], ctx->copies[1], ctx->copies[2], ctx->copies[3], ctx->tile_off, ctx->coef, ctx->keff, ctx->d_prefix, ctx->shell_tab, ctx->hist, ctx->cross, ctx->blocks_ws, ctx->feat, ctx->x_trial, ctx->x16, ctx->p16, ctx->t16, ctx->s, ctx->dF};
     for (void* b : bufs)
         if (b) cudaFree(b);
     if (ctx->ev0) cudaEventDestroy(ctx->ev0);

@@ -124,3 +124,33 @@ def test_first_calls_leave_a_capture_on_another_stream_alone():
     graph.replay()
     torch.cuda.synchronize()
     assert y.tolist() == [2.0] * 4
+
+
+def test_growing_the_workspace_does_not_wait_for_marches_in_flight():
+    """The diagonal needs more of the workspace than the renders before it; the
+    call returns while they run (calls are asynchronous)."""
+    import torch
+    ctx, xs = _context()
+    out, diag = empty(3 * ctx.n_rays), empty(xs[0].numel())
+    _context()[0].diag_jtj(xs[0], diag)   # its kernels loaded: a first launch may wait for that
+    torch.cuda.synchronize()
+    ctx.render(xs[0], out)
+    torch.cuda.synchronize()
+    for _ in range(300):
+        ctx.render(xs[0], out)
+    done = torch.cuda.Event()
+    done.record()
+    ctx.diag_jtj(xs[0], diag)
+    early = not done.query()
+    torch.cuda.synchronize()
+    assert early
+    again = empty(xs[0].numel())
+    ctx.diag_jtj(xs[0], again)
+    ap, jp = empty(xs[0].numel()), empty(3 * ctx.n_rays)
+    ctx.apply_normal(xs[0], xs[0], ap)
+    ctx.jvp(xs[0], xs[0], jp)
+    torch.cuda.synchronize()
+    # the same sums in another order of their binary32 additions
+    assert float((again - diag).norm() / diag.norm()) < 1e-5
+    dot = float((xs[0].double() * ap.double()).sum())
+    assert abs(dot - float(jp.double().square().sum())) < 1e-5 * dot
