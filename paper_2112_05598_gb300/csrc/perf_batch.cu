@@ -169,8 +169,14 @@ bool copies_ready(perf_batch* b, cudaStream_t st) {
     if (e == cudaSuccess && !b->pcopy) e = cudaMalloc(&b->pcopy, 16 * ng);
     if (e == cudaSuccess && !b->sigma8) e = cudaMalloc(&b->sigma8, 32 * nv);
     if (e == cudaSuccess && !b->diag2) e = cudaMalloc(&b->diag2, sizeof(float2) * (size_t)(b->n_params / 4));
-    if (e != cudaSuccess) {
+    if (e != cudaSuccess) {   // not enough memory: none is held
         cudaGetLastError();
+        void* made[] = {b->xcopy, b->pcopy, b->sigma8, b->diag2};
+        for (void* q : made)
+            if (q) cudaFree(q);
+        b->xcopy = b->pcopy = nullptr;
+        b->sigma8 = nullptr;
+        b->diag2 = nullptr;
         return false;
     }
     std::vector<perf::GatherDst> dst(b->n);
