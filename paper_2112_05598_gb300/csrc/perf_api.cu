@@ -1187,6 +1187,7 @@ static void set_tiling(perf_ctx* ctx, int tw) {
     d.tiles_x = (d.W + d.tile_w - 1) / d.tile_w;
     d.tiles_y = (d.H + d.tile_h - 1) / d.tile_h;
     d.n_tiles = ctx->n_rays > 0 ? (long long)d.tiles_x * d.tiles_y * d.n_cams : 0;
+    d.spread = perf::spread_of(d.n_tiles);
 }
 
 static perf_status autotune_impl(perf_ctx* ctx, const void* x, const void* p, perf_tuning* out,
