@@ -49,7 +49,11 @@ constexpr int kWarps = kThreads / 32;
 constexpr int kApplyCtas = 5;
 // the marches that read gather copies:
 constexpr int kApplyCopyCtas = 4;     // 5677; 5: 6222, 3: 6330
-constexpr int kStoreApplyCtas = 6;    // 155-157; 5: 162, 7: 176.5, 8: 163.8, 4: 164.1
+// (A p from the store strides a resident grid over the tiles, and with 6 or 4
+// CTAs its stride met the rows of small images' costly tiles: 85^3, 64 x 53 x 100,
+// 3 A p: 1370 us with 5, 1820 with 6, 1630 with 4; 134^3, 59 x 141 x 272 9130,
+// 11660, 13950; 128^3, 4 x 800^2 11944, 11945, 12459.)
+constexpr int kStoreApplyCtas = 5;
 constexpr int kDiagCopyCtas = 4;      // 6628; 3: 6752, 2: 7964
 constexpr int kVjpCopyCtas = 4;       // vjp 97^3, 5 x 333 x 251: 1005; 3: 1091, 5: 1182
 constexpr int kJvpCopyCtas = 6;       // 6809; 5: 7018, 7: 7144, 4: 7729
@@ -1427,7 +1431,8 @@ cudaError_t launch_scatter_t(const DevScene& sc, const void* x, const void* p, c
     auto fn = k_scatter<T, TP, MODE, TV, false, false, false>;
     if (sc.xcopy) fn = k_scatter<T, TP, MODE, TV, false, false, true>;
     // (not a diagonal march that also fills the store: see launch_apply_coef_t)
-    else if (sc.n_tiles - sc.tile_lo <= (MODE == 1 ? kFewTiles : kFewScatterTiles) && !coef)
+    else if (sc.n_tiles - sc.tile_lo <= (MODE == 1 ? kFewTiles : MODE == 2 ? kFewDiagTiles : kFewScatterTiles) &&
+             !coef)
         fn = k_scatter<T, TP, MODE, TV, false, false, false, MODE == 1 ? kAheadJvp : kAheadScatter>;
     if constexpr (MODE == 1) {   // A p: the counting instantiation when instrumented
         if (sc.red_count) fn = k_scatter<T, TP, MODE, TV, true, false, false>;
@@ -1500,11 +1505,13 @@ cudaError_t launch_apply_coef_t(const DevScene& sc, const void* p, const float* 
                        : (sc.red_count ? k_apply_coef<TP, true, false, false>
                           : sc.pcopy   ? k_apply_coef<TP, false, false, true>
                                        : k_apply_coef<TP, false, false, false>);
-        // A resident grid: 151.4 against 143.7 ms for a GN step at 128^3,
-    // 12 x 800^2, in march_grid's order, but a solve's last residuals and barely
-    // observed parameters follow the order of A p's additions, which a resident
-    // grid keeps from call to call; likewise for the diagonal march of a solve.
-    // (One-warp CTAs at 32^3: residual ratio R_17 / R_16 0.845 against 0.826.)
+    // A resident grid: 151 against 144 ms for a GN step at 128^3, 12 x 800^2, in
+    // march_grid's order.  Neither fixes the order of A p's additions, but the
+    // resident one varies less from run to run, and a solve's barely observed
+    // parameters magnify it: x after that step differed from earlier builds' by
+    // more than four times their own run-to-run difference in 3 of 10 runs in
+    // march_grid's order, in 0 of 8 resident; likewise for the diagonal march of a
+    // solve.  (One-warp CTAs at 32^3: residual ratio R_17 / R_16 0.845 against 0.826.)
     const int blocks = grid_blocks((const void*)fn, sc.n_tiles - sc.tile_lo, sc.cap_per_sm);
     fn<<<blocks, kThreads, 0, st>>>(
         sc, static_cast<const TP*>(p), reinterpret_cast<const float4*>(coef), tile_off, out, pap);

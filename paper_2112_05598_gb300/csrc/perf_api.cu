@@ -79,10 +79,11 @@ struct perf_ctx {
     // gather copies of the march in hand (see GatherKey in perf_device.cuh): of
     // x, of the vector J acts on, and x's opacity records.  Every use waits for
     // copy_ev, recorded behind the last one (CopyUse).
-    // Allocated as calls need them (CopyNeed), a call's missing parts together,
+    // Allocated as calls need them (parts_of), a call's missing parts together,
     // and kept: growing frees nothing, which would wait for the marches in flight.
     void* copies[4] = {nullptr, nullptr, nullptr, nullptr};
-    int copies_made = 0;        // parts, in CopyNeed's order
+    int copies_made = 0;        // parts: xcopy, sigma8, diag2, pcopy
+    double samples_per_ray = 0.0;   // grid samples of a mean ray (mean_samples)
     float4 *xcopy = nullptr, *pcopy = nullptr;
     float* sigma8 = nullptr;
     float2* diag2 = nullptr;    // packed sums of the diagonal march, n / 4 blocks
@@ -317,23 +318,73 @@ perf_status ensure_shells(perf_ctx* ctx, cudaStream_t st) {
         if (ps_ != PERF_OK) return ps_;                 \
     } while (0)
 
-// What a march needs beside x's copy.
-enum CopyNeed {
-    kNeedX = 0,
-    kNeedSigma = 1,     // x's opacity records
-    kNeedDiag = 2,      // and the packed diagonal
-    kNeedP = 3          // and the copy of the vector J acts on
+// Grid samples of a mean ray: 128 pixels, evenly apart, of at most 8 cameras.
+double mean_samples(const perf_scene& sc, const perf_cameras& cams, int max_samples) {
+    const double step = 2.0 / sc.grid_res;
+    const int nu = (int)std::fmin(32.0, std::fmax(4.0, std::sqrt(128.0 * cams.width / cams.height))), nv = 128 / nu;
+    double sum = 0.0;
+    long long rays = 0;
+    const int every = (cams.n_cams + 7) / 8;
+    for (int c = 0; c < cams.n_cams; c += every) {
+        const float* M = cams.c2w + 12 * c;
+        for (int i = 0; i < nu * nv; ++i, ++rays) {
+            const double u = ((i % nu + 0.5) / nu - 0.5) * cams.width / cams.focal[c],
+                         v = -((i / nu + 0.5) / nv - 0.5) * cams.height / cams.focal[c];
+            double lo = 0.0, hi = INFINITY, n2 = 0.0;
+            for (int a = 0; a < 3; ++a) {
+                const double d = M[4 * a] * u + M[4 * a + 1] * v - M[4 * a + 2], o = M[4 * a + 3];
+                const double t0 = (-1.0 - o) / d, t1 = (1.0 - o) / d;
+                lo = std::fmax(lo, std::fmin(t0, t1));
+                hi = std::fmin(hi, std::fmax(t0, t1));
+                n2 += d * d;
+            }
+            if (hi > lo) sum += std::fmin(std::sqrt(n2) * (hi - lo) / step + 0.5, (double)max_samples);
+        }
+    }
+    return rays ? sum / (double)rays : 0.0;
+}
+
+// The marches of x, by what they need of the workspace: x's copy, also its
+// opacity records, also the packed diagonal, also the copy of the vector J acts on.
+enum March { kForward, kVjp, kDiag, kJvp, kApply };
+int parts_of(March m) { return m >= kJvp ? 4 : (int)m + 1; }
+
+// When a march reads gather copies: at least so many samples a voxel and in all,
+// on a grid at least so large.  A copy costs 16 to 64 bytes of traffic a voxel and
+// a launch, and what the gathers from it save grows with the grid's bytes: an
+// image's gathers from a grid that the L1s nearly hold gain nothing.  us a call,
+// without / with copies:
+//   image FP32 128^3 10 x 800^2 2843 / 2525 (235 samples a voxel), 64^3 5 x 800^2
+//   618 / 676, 93^3 7 x 165 x 165 (25 a voxel) 160 / 180;
+//   BF16 256^3 4 x 800^2 2542 / 2252 (21), 128^3 4 x 800^2 1010 / 1011;
+//   J p FP32 128^3 4 x 800^2 3022 / 2103 (84), 129^3 690 x 112 (4) 158 / 190;
+//   J^T v 128^3 4 x 800^2 4609 / 3970, BF16 121^3 65 x 676 (0.2) 197 / 258;
+//   diagonal 128^3 4 x 800^2 7912 / 6873, 62^3 2 x 69 x 519 (3) 193 / 236;
+//   A p 128^3 4 x 800^2 6577 / 5525, BF16 6031 / 5538, 152^3 190 x 796 (0.8) 406 / 602.
+// Over 1100 drawn calls of 24^3 to 256^3 the lines below take 0.80 of the time
+// before copies existed; 0.3 samples a voxel for all of them took 0.85.
+struct CopyRule {
+    int G;
+    double per_voxel, samples;
+};
+constexpr CopyRule kCopyRule[5][2] = {   // FP32, BF16
+    {{100, 32, 0}, {150, 16, 0}},        // image, residual, F
+    {{0, 2, 1e6}, {0, 8, 4e6}},          // J^T v
+    {{0, 4, 2e6}, {0, 2, 2e6}},          // diagonal
+    {{0, 8, 1e6}, {0, 32, 8e6}},         // J p
+    {{0, 2, 1e6}, {0, 16, 2e7}},         // A p
 };
 
-// Whether the marches of x read gather copies (0.6 G samples a ray, a little
-// above the mean chord through the grid).
-bool copies_pay(const perf_ctx* ctx, CopyNeed what) {
-    const double samples = 0.6 * (double)ctx->ds.G * (double)ctx->n_rays;
-    const long long few = what == kNeedX   ? perf::kMidTiles
-                          : what == kNeedP ? perf::kFewTiles
-                                           : perf::kFewScatterTiles;
-    return ctx->ds.n_tiles > few &&
-           samples >= perf::kCopyRatio * (double)ctx->ds.n_vox;
+double samples_of(const perf_ctx* ctx) { return ctx->samples_per_ray * (double)ctx->n_rays; }
+
+bool copies_pay(const perf_ctx* ctx, March m) {
+    const CopyRule& r = kCopyRule[m][ctx->scene.dtype == PERF_BF16];
+    const long long few = m == kForward ? perf::kMidTiles
+                          : m >= kJvp   ? perf::kFewTiles
+                                        : perf::kFewScatterTiles;
+    const double samples = samples_of(ctx);
+    return ctx->ds.n_tiles > few && ctx->ds.G >= r.G && samples >= r.samples &&
+           samples >= r.per_voxel * (double)ctx->ds.n_vox;
 }
 
 // A call's use of the gather copies on st: from take() on, whatever way the
@@ -364,10 +415,9 @@ struct CopyUse {
 };
 
 // Room for the gather copies of a march on use.st, free of earlier calls' use;
-// false: the march gathers from x and p themselves -- few samples, no memory,
-// or a stream under capture, whose graph would keep the workspace.
-bool copies_ready(perf_ctx* ctx, CopyNeed what, CopyUse& use) {
-    if (!copies_pay(ctx, what)) return false;
+// false: the march gathers from x and p themselves -- no memory, or a stream
+// under capture, whose graph would keep the workspace.
+bool copies_room(perf_ctx* ctx, int parts, CopyUse& use) {
     const cudaStream_t st = use.st;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
@@ -375,25 +425,25 @@ bool copies_ready(perf_ctx* ctx, CopyNeed what, CopyUse& use) {
         return false;
     }
     const perf::BesideCapture beside;
-    if (ctx->copies_made <= what) {
+    if (ctx->copies_made < parts) {
         // the parts that earlier calls did not need, in one allocation
         const size_t ng = sizeof(float4) * (size_t)perf::gather_size(ctx->ds.G);
         const size_t bytes[4] = {ng, 8 * sizeof(float) * (size_t)ctx->ds.n_vox,
                                  sizeof(float2) * (((size_t)ctx->n / 4 + 1) / 2 * 2), ng};
         size_t need = 0;
-        for (int q = ctx->copies_made; q <= what; ++q) need += bytes[q];
+        for (int q = ctx->copies_made; q < parts; ++q) need += bytes[q];
         char* at = nullptr;
         if (cudaMalloc(&at, need) != cudaSuccess) {
             cudaGetLastError();
             return false;
         }
         ctx->copies[ctx->copies_made] = at;
-        for (; ctx->copies_made <= what; ++ctx->copies_made) {
+        for (; ctx->copies_made < parts; ++ctx->copies_made) {
             void* part = at;
             switch (ctx->copies_made) {
-                case kNeedX: ctx->xcopy = static_cast<float4*>(part); break;
-                case kNeedSigma: ctx->sigma8 = static_cast<float*>(part); break;
-                case kNeedDiag: ctx->diag2 = static_cast<float2*>(part); break;
+                case 0: ctx->xcopy = static_cast<float4*>(part); break;
+                case 1: ctx->sigma8 = static_cast<float*>(part); break;
+                case 2: ctx->diag2 = static_cast<float2*>(part); break;
                 default: ctx->pcopy = static_cast<float4*>(part);
             }
             at += bytes[ctx->copies_made];
@@ -424,6 +474,16 @@ int solver_spread(const perf_ctx* ctx) {
     return scatter_spread(ctx);
 }
 
+// Whether they read copies: by the diagonal march, which runs in every step, and
+// where an image has 3 pixels a voxel column -- with fewer a warp's rays share
+// no lines, and A p from the store gains nothing from p's copy (us a step's 3 A p
+// without / with: 85^3, 53 x 100 1270 / 1370, 134^3, 141 x 272 8875 / 9130; 96^3,
+// 200^2 2530 / 2080, 64^3, 128^2 2640 / 2400, 128^3, 800^2 12290 / 11940).
+bool solver_copies(const perf_ctx* ctx) {
+    const perf::DevScene& d = ctx->ds;
+    return solver_spread(ctx) && (double)d.W * d.H >= 3.0 * d.G * d.G && copies_pay(ctx, kDiag);
+}
+
 // d for a solve's scatters without copies, resident where the spread order is
 // left for the plain one.
 void plain_scatter(const perf_ctx* ctx, perf::DevScene& d) {
@@ -434,16 +494,32 @@ void plain_scatter(const perf_ctx* ctx, perf::DevScene& d) {
     if (ctx->ds.spread && !d.spread && d.cap_per_sm == 0) d.cap_per_sm = kResident;
 }
 
-// d = the context's scene with the gather copies of x (and, with kNeedP, of p
-// in type p_dtype), made on use.st, where they pay.
-perf_status gather_copies(perf_ctx* ctx, const void* x, const void* p, int p_dtype, CopyNeed what,
+// Whether very many pixels of an image look through each voxel: tiles side by
+// side then add to the same few voxels, and on CTAs placed in order they do so
+// together.  A resident grid's drift apart (diagonal, us, in order / resident:
+// 28^3, 533 x 283 (192 pixels a voxel column) 7416 / 4449; 64^3, 800^2 (156) 4984
+// / 4054; 36^3, 354 x 208 (57) 4050 / 2937; below 32 in order by 2 to 12%; J^T v
+// and A p, whose reductions are fewer, 5% either way above 128, and by 1.4 to 1.7
+// at worst in order).
+bool crowded(const perf_ctx* ctx) {
+    const perf::DevScene& d = ctx->ds;
+    return (double)d.W * d.H >= 100.0 * d.G * d.G || (d.spread && !scatter_spread(ctx));
+}
+
+// d = the context's scene for march m with the gather copies of x (and of p, in
+// type p_dtype), made on use.st, if `pay`.
+perf_status gather_copies(perf_ctx* ctx, const void* x, const void* p, int p_dtype, March m, bool pay,
                           CopyUse& use, perf::DevScene& d) {
     d = ctx->ds;
-    if (what != kNeedX) d.spread = scatter_spread(ctx);
-    if (!copies_ready(ctx, what, use)) return PERF_OK;
+    if (m != kForward && m != kJvp) {
+        d.spread = scatter_spread(ctx);
+        if (ctx->ds.spread && !d.spread) pay = false;
+        if (d.cap_per_sm == 0 && crowded(ctx)) d.cap_per_sm = kResident;
+    }
+    const int parts = parts_of(m);
+    if (!pay || !copies_room(ctx, parts, use)) return PERF_OK;
     CK(perf::launch_gather_copy(d.n_vox, d.G, ctx->scene.dtype, x, ctx->xcopy,
-                                what >= kNeedSigma ? ctx->sigma8 : nullptr, use.st, p_dtype, p,
-                                ctx->pcopy));
+                                parts > 1 ? ctx->sigma8 : nullptr, use.st, p_dtype, p, ctx->pcopy));
     d.xcopy = ctx->xcopy;
     d.pcopy = p ? ctx->pcopy : nullptr;
     d.sigma8 = ctx->sigma8;
@@ -464,12 +540,13 @@ perf_status diag_march(perf_ctx* ctx, const perf::DevScene& d, const void* x, co
     return PERF_OK;
 }
 
-#define COPIES(ctx, x, p, what, st, d)                                            \
-    perf::DevScene d;                                                             \
-    CopyUse use_(ctx, st);                                                        \
-    do {                                                                          \
-        const perf_status ps_ = gather_copies(ctx, x, p, PERF_F32, what, use_, d); \
-        if (ps_ != PERF_OK) return ps_;                                           \
+#define COPIES(ctx, x, p, march, st, d)                                                 \
+    perf::DevScene d;                                                                   \
+    CopyUse use_(ctx, st);                                                              \
+    do {                                                                                \
+        const perf_status ps_ =                                                         \
+            gather_copies(ctx, x, p, PERF_F32, march, copies_pay(ctx, march), use_, d); \
+        if (ps_ != PERF_OK) return ps_;                                                 \
     } while (0)
 
 void t_begin(perf_ctx* c, int k, cudaStream_t st) {
@@ -590,6 +667,7 @@ perf_status perf_create(perf_ctx** out, const perf_scene* sc, const perf_cameras
     d.n_tiles = (long long)d.tiles_x * d.tiles_y * cams->n_cams;
     if (ctx->n_rays == 0) d.n_tiles = 0;
     d.spread = perf::spread_of(d.n_tiles);
+    if (ctx->n_rays > 0) ctx->samples_per_ray = mean_samples(*sc, *cams, opts->max_samples);
     d.max_samples = opts->max_samples;
     d.jitter = opts->jitter;
     d.aux = opts->aux;
@@ -672,7 +750,7 @@ perf_status perf_render(perf_ctx* ctx, const void* x, float* rgb_out, float* T_o
     if (ctx->n_rays == 0) return PERF_OK;
     if (bad_ptr(x) || bad_ptr(rgb_out)) return fail(ctx, PERF_ERR_INVALID_ARG, "render: NULL x or rgb_out");
     SHELLS(ctx, S(stream));
-    COPIES(ctx, x, nullptr, kNeedX, S(stream), d);
+    COPIES(ctx, x, nullptr, kForward, S(stream), d);
     CK(perf::launch_forward(d, ctx->scene.dtype, x, nullptr, rgb_out, T_out, nullptr, 0, S(stream)));
     return PERF_OK;
 }
@@ -685,7 +763,7 @@ perf_status perf_residual(perf_ctx* ctx, const void* x, const void* target, void
     if (ctx->n_rays == 0) return PERF_OK;
     if (bad_ptr(x) || bad_ptr(target)) return fail(ctx, PERF_ERR_INVALID_ARG, "residual: NULL x or target");
     SHELLS(ctx, S(stream));
-    COPIES(ctx, x, nullptr, kNeedX, S(stream), d);
+    COPIES(ctx, x, nullptr, kForward, S(stream), d);
     CK(perf::launch_forward(d, ctx->scene.dtype, x, target, r_out, nullptr, F_out,
                             r_out ? 1 : 2, S(stream)));
     return PERF_OK;
@@ -696,7 +774,7 @@ perf_status perf_jvp(perf_ctx* ctx, const void* x, const float* p, float* jp_out
     if (ctx->n_rays == 0) return PERF_OK;
     if (bad_ptr(x) || bad_ptr(p) || bad_ptr(jp_out)) return fail(ctx, PERF_ERR_INVALID_ARG, "jvp: NULL pointer");
     SHELLS(ctx, S(stream));
-    COPIES(ctx, x, p, kNeedP, S(stream), d);
+    COPIES(ctx, x, p, kJvp, S(stream), d);
     CK(perf::launch_jvp(d, ctx->scene.dtype, x, p, PERF_F32, jp_out, S(stream)));
     return PERF_OK;
 }
@@ -709,7 +787,7 @@ perf_status perf_vjp(perf_ctx* ctx, const void* x, const float* v, float* out, i
     if (ctx->n_rays == 0) return PERF_OK;
     if (bad_ptr(x) || bad_ptr(v)) return fail(ctx, PERF_ERR_INVALID_ARG, "vjp: NULL x or v");
     SHELLS(ctx, S(stream));
-    COPIES(ctx, x, nullptr, kNeedSigma, S(stream), d);
+    COPIES(ctx, x, nullptr, kVjp, S(stream), d);
     CK(perf::launch_scatter(d, ctx->scene.dtype, 0, x, nullptr, PERF_F32, v, out, nullptr,
                             nullptr, S(stream)));
     return PERF_OK;
@@ -728,7 +806,7 @@ perf_status perf_diag_jtj(perf_ctx* ctx, const void* x, const void* r, float* di
     }
     if (bad_ptr(x)) return fail(ctx, PERF_ERR_INVALID_ARG, "diag_jtj: NULL x");
     SHELLS(ctx, S(stream));
-    COPIES(ctx, x, nullptr, kNeedDiag, S(stream), d);
+    COPIES(ctx, x, nullptr, kDiag, S(stream), d);
     const perf_status ps = diag_march(ctx, d, x, r, diag_out, grad_out, nullptr, nullptr, nullptr, S(stream));
     return ps;
 }
@@ -742,7 +820,7 @@ perf_status perf_apply_normal(perf_ctx* ctx, const void* x, const float* p, floa
     if (ctx->n_rays == 0) return PERF_OK;
     if (bad_ptr(x) || bad_ptr(p)) return fail(ctx, PERF_ERR_INVALID_ARG, "apply_normal: NULL x or p");
     SHELLS(ctx, S(stream));
-    COPIES(ctx, x, p, kNeedP, S(stream), d);
+    COPIES(ctx, x, p, kApply, S(stream), d);
     CK(perf::launch_scatter(d, ctx->scene.dtype, 1, x, p, PERF_F32, nullptr, ap_out, nullptr,
                             pap_out, S(stream)));
     return PERF_OK;
@@ -887,7 +965,7 @@ perf_status perf_pcg_step(perf_ctx* ctx, const void* x, int32_t* done_out, void*
     CopyUse use(ctx, S(stream));
     if (solver_spread(ctx)) {
         st = gather_copies(ctx, x, bf ? static_cast<const void*>(ctx->p16) : ctx->p, ctx->scene.dtype,
-                           kNeedP, use, d);
+                           kApply, copies_pay(ctx, kApply), use, d);
     } else {
         d = ctx->ds;
         plain_scatter(ctx, d);
@@ -958,15 +1036,11 @@ perf_status perf_gn_solve(perf_ctx* ctx, float* x, const void* target, int32_t n
         // the step's marches of x read its gather copy, the A p that of p
         perf::DevScene ds = ctx->ds;
         const int spread = solver_spread(ctx);
-        const bool copies = ctx->n_rays > 0 && copies_ready(ctx, spread ? kNeedP : kNeedX, use);
-        const bool scatter_copies = copies && spread;
+        const bool scatter_copies = solver_copies(ctx) && copies_room(ctx, 4, use);
+        const bool copies = copies_pay(ctx, kForward) && copies_room(ctx, 1, use);
         if (copies) ds.xcopy = ctx->xcopy;
-        if (scatter_copies) {
-            ds.sigma8 = ctx->sigma8;
-            ds.diag2 = ctx->diag2;
-        }
         t_begin(ctx, PERF_T_RESIDUAL, st);
-        if (copies)
+        if (copies || scatter_copies)
             CK(perf::launch_gather_copy(ds.n_vox, ds.G, ctx->scene.dtype, xm, ctx->xcopy,
                                         scatter_copies ? ctx->sigma8 : nullptr, st));
         if (ctx->n_rays > 0)
@@ -994,7 +1068,19 @@ perf_status perf_gn_solve(perf_ctx* ctx, float* x, const void* target, int32_t n
         // canonical order
         perf::DevScene dl = ds;
         dl.spread = spread;
-        if (!scatter_copies) plain_scatter(ctx, dl);
+        int diag_cap = 0;
+        if (scatter_copies) {
+            dl.xcopy = ctx->xcopy;
+            dl.sigma8 = ctx->sigma8;
+            dl.diag2 = ctx->diag2;
+            if (dl.cap_per_sm == 0 && crowded(ctx)) dl.cap_per_sm = kResident;
+            // (its 4 CTAs an SM stride 2432 tiles, which in images that mostly miss
+            // the grid met the costly rows again and again: 127^3, 16 x 79 x 648,
+            // 2000 us with 4, 1100 with 3; elsewhere 4 are 2% faster)
+            if (dl.cap_per_sm == 0 && ctx->samples_per_ray < 0.25 * ds.G) diag_cap = 3;
+        } else {
+            plain_scatter(ctx, dl);
+        }
         perf::set_layout(dl, (use_coef && ctx->coef_tiles >= ctx->ds.n_tiles &&
                               o.precond != PERF_PRECOND_BLOCK4) ? ctx->brick_s : 0);
         dl.keff = use_coef ? ctx->keff : nullptr;
@@ -1002,7 +1088,9 @@ perf_status perf_gn_solve(perf_ctx* ctx, float* x, const void* target, int32_t n
         if (scatter_copies && dl.lay_s == 0) dl.pcopy = ctx->pcopy;
         const int4 lay = perf::layout_of(dl);
         t_begin(ctx, PERF_T_DIAG, st);
-        ps = diag_march(ctx, dl, xm, ctx->r, ctx->diag, ctx->grad, need_cross ? ctx->cross : nullptr,
+        perf::DevScene dd = dl;
+        if (diag_cap) dd.cap_per_sm = diag_cap;
+        ps = diag_march(ctx, dd, xm, ctx->r, ctx->diag, ctx->grad, need_cross ? ctx->cross : nullptr,
                         use_coef ? ctx->coef : nullptr, use_coef ? ctx->tile_off : nullptr, st);
         if (ps != PERF_OK) return ps;
         t_end(ctx, PERF_T_DIAG, st);
@@ -1039,7 +1127,7 @@ perf_status perf_gn_solve(perf_ctx* ctx, float* x, const void* target, int32_t n
         int evals = 0;
         bool accept = false;
         for (int pass = 0; pass < 2; ++pass) {
-            if (pass == 1 && scatter_copies && dl.coef_tiles < dl.n_tiles)   // the line search's trial points took its place
+            if (pass == 1 && copies && scatter_copies && dl.coef_tiles < dl.n_tiles)   // the line search's trial points took its place
                 CK(perf::launch_gather_copy(ds.n_vox, ds.G, ctx->scene.dtype, xm, ctx->xcopy, nullptr, st));
             for (int attempt = 0; attempt < 2; ++attempt) {
                 ps = ensure_hist(ctx, o.pcg_iters);
@@ -1205,7 +1293,7 @@ static perf_status autotune_impl(perf_ctx* ctx, const void* x, const void* p, pe
     // the solver's A p gathers from copies where they pay: so does the tuner's
     perf::DevScene dc;
     CopyUse use(ctx, st);
-    ps = gather_copies(ctx, x, pp, ctx->scene.dtype, kNeedP, use, dc);
+    ps = gather_copies(ctx, x, pp, ctx->scene.dtype, kApply, solver_copies(ctx), use, dc);
     if (ps != PERF_OK) return ps;
     auto scene = [&]() {
         perf::DevScene d = ctx->ds;
@@ -1394,7 +1482,7 @@ perf_status perf_diag_cross(perf_ctx* ctx, const void* x, float* diag_out, float
     }
     if (bad_ptr(x)) return fail(ctx, PERF_ERR_INVALID_ARG, "diag_cross: NULL x");
     SHELLS(ctx, S(stream));
-    COPIES(ctx, x, nullptr, kNeedDiag, S(stream), d);
+    COPIES(ctx, x, nullptr, kDiag, S(stream), d);
     const perf_status ps = diag_march(ctx, d, x, nullptr, diag_out, nullptr, cross_out, nullptr, nullptr, S(stream));
     return ps;
 }
@@ -1419,8 +1507,10 @@ perf_status perf_adam_step(perf_ctx* ctx, float* x, const void* target, float* m
     if (ctx->n_rays > 0) {
         SHELLS(ctx, st);
         // r = H^ - C and F, then g = J^T r (Section "Update step": the gradient)
-        COPIES(ctx, x, nullptr, kNeedSigma, st, d);
-        CK(perf::launch_forward(d, PERF_F32, x, target, ctx->r, nullptr, ctx->dF, 1, st));
+        COPIES(ctx, x, nullptr, kVjp, st, d);
+        perf::DevScene f = d;
+        if (!copies_pay(ctx, kForward)) f.xcopy = nullptr;
+        CK(perf::launch_forward(f, PERF_F32, x, target, ctx->r, nullptr, ctx->dF, 1, st));
         CK(perf::launch_scatter(d, PERF_F32, 0, x, nullptr, PERF_F32, ctx->r, ctx->grad, nullptr,
                                 nullptr, st));
     }
@@ -1521,7 +1611,7 @@ perf_status perf_render_threshold(perf_ctx* ctx, const void* x, float min_opacit
     if (ctx->n_rays == 0) return PERF_OK;
     if (bad_ptr(x) || bad_ptr(rgb_out)) return fail(ctx, PERF_ERR_INVALID_ARG, "render_threshold: NULL x or rgb_out");
     SHELLS(ctx, S(stream));
-    COPIES(ctx, x, nullptr, kNeedX, S(stream), d);
+    COPIES(ctx, x, nullptr, kForward, S(stream), d);
     CK(perf::launch_forward(d, ctx->scene.dtype, x, nullptr, rgb_out, T_out, nullptr, 0, S(stream),
                             min_opacity));
     return PERF_OK;

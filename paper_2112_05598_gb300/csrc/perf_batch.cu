@@ -144,8 +144,7 @@ perf_status apply_tiling(perf_batch* b, int tw) {
 
 // Gather copies (see GatherKey in perf_device.cuh) of every scene's grid: of the
 // x in hand, of p, and the opacity records of x.  Whether a march reads them:
-// as copies_pay in perf_api.cu, over the batch; made once, and not on a stream
-// under capture.
+// kCopyRatio, over the batch; made once, and not on a stream under capture.
 bool copies_ready(perf_batch* b, cudaStream_t st) {
     double samples = 0.0, voxels = 0.0;
     for (const BatchItem& it : b->items) {

@@ -134,11 +134,12 @@ inline void count_launch(unsigned long long k = 1) { __atomic_fetch_add(&g_launc
 // lane order: J^T v 32^3, 12 x 64^2 (1536 tiles) 75 / 88, 30^3, 103 x 417 (1365)
 // 67 / 60.
 constexpr long long kFewTiles = 152 * 12, kMidTiles = 152 * 28, kFewScatterTiles = 152 * 10 - 1;
-// A march gathers from copies when its samples are at least this many per
-// voxel.  A copy moves 32 bytes a voxel (the opacity records up to 48 more) in
-// one launch; on a 128^3 grid with 3 shells, us a call without / with copies:
-// render 121 / 111, jvp 414 / 356, A p 543 / 413 at 0.37 samples a voxel
-// (100^2 rays), 161 / 134, 473 / 323, 866 / 623 at 5.9 (400^2).
+// The diagonal's groups of two leave 8 warps an SM room (255 registers): 90^3, 283
+// x 166 (1512 tiles) 220 / 284 us, 204^3 BF16, 231 x 179 (1305) 602 / 791; up to 8
+// an SM 5% the other way.
+constexpr long long kFewDiagTiles = 152 * 8;
+// The marches of a batch gather from copies when its scenes have at least this
+// many samples per voxel together (a single scene's: kCopyRule in perf_api.cu).
 constexpr double kCopyRatio = 0.3;
 // Gather copies of the n_vox grid voxels of x (and of p, if given) and x's
 // opacity records (sig, may be null): see GatherKey (gather_size(G) voxels per
