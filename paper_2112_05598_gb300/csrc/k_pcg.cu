@@ -18,7 +18,7 @@
 //           beta = rho'^T z' / rho^T z                               [1 thread]
 //   dir   : p = z + beta p
 // Bytes per parameter and iteration: update 20 read + 12 written, dir 12
-// read + 4 written (48; BF16 scenes write 2 more, a gather copy of p 4 or 2).
+// read + 4 written (48; BF16 scenes write 2 more, a gather copy of p 4).
 // M^-1 is Jacobi (z_j = rho_j / d_j, 0 where d_j <= 1e-30) or, where 4x4 blocks
 // are given for the grid voxels, z_v = P_v rho_v per voxel.
 #include <cuda_bf16.h>
@@ -118,9 +118,7 @@ __device__ __forceinline__ void store_p(float4* p, __nv_bfloat16* p16, long long
     if (p16) store_bf16x4(p16, v, f);
     const long long u = v - g.first;
     if (g.copy && u < g.nv) {
-        const int at = gather_place((int)u, g.G);
-        auto r = [&](float a) { return g.bf16 ? __bfloat162float(__float2bfloat16_rn(a)) : a; };
-        g.copy[at] = make_float4(r(f.x), r(f.y), r(f.z), r(f.w));
+        g.copy[gather_place((int)u, g.G)] = f;
     }
 }
 

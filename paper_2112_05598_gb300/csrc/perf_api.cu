@@ -860,9 +860,8 @@ cudaError_t apply_arrays(perf_ctx* ctx, const perf::DevScene& d, const void* x, 
 }
 
 // Where the PCG kernels also write p for the A p's gathers: the copy d names.
-perf::GatherDst gather_dst(const perf_ctx* ctx, const perf::DevScene& d) {
-    return perf::GatherDst{const_cast<float4*>(d.pcopy), 0, d.n_vox, d.G,
-                           ctx->scene.dtype == PERF_BF16 ? 1 : 0};
+perf::GatherDst gather_dst(const perf::DevScene& d) {
+    return perf::GatherDst{const_cast<float4*>(d.pcopy), 0, d.n_vox, d.G};
 }
 
 // One Algorithm 2 iteration on the context workspace with diagonal `diag`
@@ -891,7 +890,7 @@ perf_status pcg_iter(perf_ctx* ctx, const void* x, const float* diag, const floa
                                ctx->s, st));
     CK(perf::launch_pcg_finish(ctx->s, st));
     CK(perf::launch_pcg_dir(ctx->n, ctx->rho, diag, B, ctx->n_block, ctx->p, ctx->p16, ctx->s, st,
-                            gather_dst(ctx, d0)));
+                            gather_dst(d0)));
     t_end(ctx, PERF_T_VECTOR, st);
     return PERF_OK;
 }
@@ -1135,7 +1134,7 @@ perf_status perf_gn_solve(perf_ctx* ctx, float* x, const void* target, int32_t n
                 CK(perf::launch_pcg_begin(ctx->n, ctx->grad, ctx->diag, ctx->delta, ctx->rho, ctx->p,
                                           ctx->p16, ctx->Ap, ctx->s, o.pcg_iters, o.pcg_fixed,
                                           o.pcg_eps_rel, o.pcg_stall, B, nB, st, ctx->hist,
-                                          ctx->hist_cap, gather_dst(ctx, dl)));
+                                          ctx->hist_cap, gather_dst(dl)));
                 if (o.pcg_fixed && ctx->pcg_graph_on && !ctx->timing && o.pcg_iters > 1) {
                     // one graph for the whole loop (no per-kernel launch work on the host)
                     ps = pcg_graph_run(ctx, xm, B, use_coef, dl, o.pcg_iters, st);

@@ -186,7 +186,7 @@ bool copies_ready(perf_batch* b, cudaStream_t st) {
         d.pcopy = b->pcopy + ng;
         d.sigma8 = b->sigma8 + 8 * nv;
         d.diag2 = b->diag2 + b->items[i].x_off / 4;
-        dst[i] = perf::GatherDst{b->pcopy + ng, b->items[i].x_off / 4, d.n_vox, d.G, 0};
+        dst[i] = perf::GatherDst{b->pcopy + ng, b->items[i].x_off / 4, d.n_vox, d.G};
         ng += (size_t)perf::gather_size(d.G);
         nv += (size_t)d.n_vox;
     }

@@ -272,16 +272,8 @@ template <> struct Store<__nv_bfloat16> {
     }
 };
 
-__device__ __forceinline__ float4 lerp4(float4 a, float4 b, float t) {
-    return make_float4(fmaf(t, b.x - a.x, a.x), fmaf(t, b.y - a.y, a.y),
-                       fmaf(t, b.z - a.z, a.z), fmaf(t, b.w - a.w, a.w));
-}
-
 // Trilinear interpolation as a weighted sum of the 8 corners (corner c:
 // bit a = +1 along axis a), weights w_c = prod_a (c_a ? f_a : 1 - f_a).
-#ifndef PERF_INTERP_W
-#define PERF_INTERP_W 1
-#endif
 __device__ __forceinline__ void tri_weights(const Cell& c, float (&W)[8]) {
     const float gx[2] = {1.0f - c.fx, c.fx}, gy[2] = {1.0f - c.fy, c.fy}, gz[2] = {1.0f - c.fz, c.fz};
 #pragma unroll
@@ -315,16 +307,9 @@ __device__ __forceinline__ float4 interp_grid(const T* x, const DevScene& sc, co
     a[5] = Store<T>::ld(x, i0 + sz + 1);
     a[6] = Store<T>::ld(x, i0 + sz + sy);
     a[7] = Store<T>::ld(x, i0 + sz + sy + 1);
-#if PERF_INTERP_W
     float W[8];
     tri_weights(c, W);
     return wsum8(W, a);
-#else
-    const float4 b00 = lerp4(a[0], a[1], c.fx), b10 = lerp4(a[2], a[3], c.fx);
-    const float4 b01 = lerp4(a[4], a[5], c.fx), b11 = lerp4(a[6], a[7], c.fx);
-    const float4 c0 = lerp4(b00, b10, c.fy), c1 = lerp4(b01, b11, c.fy);
-    return lerp4(c0, c1, c.fz);
-#endif
 }
 
 // interp_grid for a vector stored in the order of a LayoutKey.
@@ -342,16 +327,9 @@ __device__ __forceinline__ float4 interp_grid_lay(const T* x, const LayoutKey& k
     a[5] = Store<T>::ld(x, x1 + y0 + z1);
     a[6] = Store<T>::ld(x, x0 + y1 + z1);
     a[7] = Store<T>::ld(x, x1 + y1 + z1);
-#if PERF_INTERP_W
     float W[8];
     tri_weights(c, W);
     return wsum8(W, a);
-#else
-    const float4 b00 = lerp4(a[0], a[1], c.fx), b10 = lerp4(a[2], a[3], c.fx);
-    const float4 b01 = lerp4(a[4], a[5], c.fx), b11 = lerp4(a[6], a[7], c.fx);
-    const float4 c0 = lerp4(b00, b10, c.fy), c1 = lerp4(b01, b11, c.fy);
-    return lerp4(c0, c1, c.fz);
-#endif
 }
 
 // --- packed binary32 pairs (FFMA2): two independent round-to-nearest

@@ -160,7 +160,6 @@ struct GatherDst {
     long long first;       // first parameter block of the system
     long long nv;          // its grid voxels
     int G;
-    int bf16;              // 1: the gathered p is BF16 (the copy holds its rounded values)
 };
 
 // While it lives, this thread's allocations are allowed beside a capture on
