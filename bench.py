@@ -67,9 +67,9 @@ APPLY_COMPULSORY_BYTES_PER_PARAM = 16
 COEF_BYTES_PER_SAMPLE = 32
 # PCG vector kernels per iteration: update reads p, A p, Delta, rho, d (20 B)
 # and writes Delta, rho, A p = 0 (12 B); direction reads rho, d, p (12 B) and
-# writes p (4 B): 48 bytes per parameter (+2 for the BF16 copy of p).  The
-# scope's count for the fused vector work is 11 n-vector passes of 4 bytes (44
-# bytes per parameter).
+# writes p (4 B): 48 bytes per parameter (+2 for the BF16 copy of p, +4 per grid
+# parameter for p's gather copy).  The scope's count for the fused vector work is
+# 11 n-vector passes of 4 bytes (44 bytes per parameter).
 VEC_BYTES_PER_PARAM = 48
 VEC_COMPULSORY_BYTES_PER_PARAM = 44
 # The residual pass streams the targets C in and the residuals r out: 12 + 12
@@ -82,6 +82,55 @@ RESIDUAL_BYTES_PER_RAY_F32 = 24
 TRAFFIC_PROFILE = os.path.join(ROOT, "profiles", "apply_coef_traffic_scale128.md")
 KERNEL_SOURCES = ("paper_2112_05598_gb300/csrc/k_march.cu",
                   "paper_2112_05598_gb300/csrc/perf_device.cuh")
+
+
+# Readers of the line keep about 3000 characters of it.
+LINE_LIMIT = 2600
+# What a longer record keeps whole, what it loses first (curves, per-step lists),
+# and what it does without, the least telling first.
+_WHOLE = ("config", "e2e", "clocks")
+_LONG = ("psnr_curve", "runs", "gn_steps", "first_system_pcg", "training")
+_OPTIONAL = ("residual_roofline", "kernel_ms_per_step", "vector_roofline", "rays_per_s", "apply_ms_per_launch",
+             "cpu_baseline", "lpc")
+
+
+def kept_line(line, limit=LINE_LIMIT):
+    """`line` within `limit` characters of JSON: the contract's keys as they are;
+    of the other records their own short values, nested numbers to 6 digits."""
+    if len(json.dumps(line)) <= limit:
+        return line
+
+    def short(v):
+        if isinstance(v, dict):
+            return {k: short(x) for k, x in v.items() if k not in _LONG}
+        if isinstance(v, float):
+            return float(f"{v:.6g}")
+        return v[:80] if isinstance(v, str) else v
+
+    out = {}
+    for k, v in line.items():
+        if k in _WHOLE or not isinstance(v, (dict, list)):
+            out[k] = v
+        elif k == "lpc":
+            out[k] = {"summary": short(v.get("summary"))}
+        elif k not in _LONG and isinstance(v, dict):
+            out[k] = short({q: x for q, x in v.items() if not isinstance(x, (dict, list))})
+            if isinstance(v.get("atomics"), dict):
+                out[k]["atomics_frac"] = short(v["atomics"].get("frac"))
+    for k in _OPTIONAL:
+        if len(json.dumps(out)) <= limit:
+            break
+        out.pop(k, None)
+    return out
+
+
+def emit(line):
+    """Prints the one line; a record that is longer goes whole to stderr first."""
+    import sys
+    kept = kept_line(line)
+    if kept is not line:
+        print("bench record: " + json.dumps(line), file=sys.stderr, flush=True)
+    print(json.dumps(kept), flush=True)
 
 
 def kernel_source_hash():
@@ -332,7 +381,7 @@ def run_reference(args, rank, world):
             "cpu_baseline": {"value": v, "unit": METRIC, "cores": os.cpu_count(),
                              "cpu": cpu_model(), "kind": "oracle", "sample": timed[0]["sample"]},
             "e2e": {"value": v, "unit": METRIC, "h2d_bytes_per_step": 0, "d2h_bytes_per_step": 0}}
-    print(json.dumps(line), flush=True)
+    emit(line)
 
 
 def _scene_config(args):
@@ -409,7 +458,7 @@ def run_conv(args, rank, world, local):
                          "hbm_frac": byts / (ms * 1e-3) / 1e9 / peaks["hbm_gbs"],
                          "kernel": "k_conv_fwd_tc (tcgen05, TMA halo staging)"}}
     if rank == 0:
-        print(json.dumps(line), flush=True)
+        emit(line)
 
 
 def lpc_study(dev, workload, n_cams=None, train_small=100, train_steps=20, train_large=8,
@@ -697,7 +746,7 @@ def run_hier(args, rank, world, local):
             "runs": runs}
     for h, _ in holds.values():
         h.close()
-    print(json.dumps(line), flush=True)
+    emit(line)
 
 
 def run_compare(args, rank, world, local):
@@ -789,7 +838,7 @@ def run_compare(args, rank, world, local):
                                                    "cube": cube["psnr_curve"][-1][1]},
                                  "shell_texels": {"equirect": "2 x 32x64", "cube": "2 x 6x16x16"},
                                  "equirect": gn, "cube": cube}}
-    print(json.dumps(line), flush=True)
+    emit(line)
 
 
 def run_batch(args, rank, world, local):
@@ -869,7 +918,7 @@ def run_batch(args, rank, world, local):
                     "d2h_bytes_per_step": int(4 * b.n_params)},
             "clocks": clk,
             "accepted_fraction": float(np.mean([s["accepted"] for st in stats for s in st]))}
-    print(json.dumps(line), flush=True)
+    emit(line)
 
 
 def rows_read_fraction(ctx):
@@ -1091,13 +1140,15 @@ def run_ours(args, rank, world, local):
                        "peak": red_peak, "unit": "lane-ops/s", "frac": red_rate / red_peak,
                        "peak_source": "perf_measure_atomic_peak (16-byte vector atomic "
                                       "microbenchmark on this GPU, measured in this run)"}
-    vb = VEC_BYTES_PER_PARAM + (2 if bf else 0)
+    vec_bytes = (VEC_BYTES_PER_PARAM + (2 if bf else 0)) * sc.n_params
+    if not bf and tuning.get("brick", 1) == 1 and samples >= 4 * sc.G ** 3:
+        vec_bytes += 4 * 4 * sc.G ** 3   # k_pcg_dir also writes p's gather copy
     vec_s = tm["vector"]["ms"] / 1000.0 / iters
     vector_roof = {"kernels": "k_pcg_update + k_pcg_finish + k_pcg_dir (per PCG iteration)",
-                   "bound": "hbm", "bytes_per_iter": vb * sc.n_params,
+                   "bound": "hbm", "bytes_per_iter": vec_bytes,
                    "ms_per_iter": vec_s * 1000.0,
-                   "achieved": vb * sc.n_params / vec_s / 1e9, "peak": hbm_peak, "unit": "GB/s",
-                   "frac": vb * sc.n_params / vec_s / 1e9 / hbm_peak,
+                   "achieved": vec_bytes / vec_s / 1e9, "peak": hbm_peak, "unit": "GB/s",
+                   "frac": vec_bytes / vec_s / 1e9 / hbm_peak,
                    "compulsory_bytes_per_iter": VEC_COMPULSORY_BYTES_PER_PARAM * sc.n_params,
                    "frac_compulsory": VEC_COMPULSORY_BYTES_PER_PARAM * sc.n_params / vec_s / 1e9
                    / hbm_peak,
@@ -1151,7 +1202,7 @@ def run_ours(args, rank, world, local):
         torch.cuda.empty_cache()
         line["lpc"] = lpc_study(dev, "ring128", train_small=100, train_steps=20, train_large=8,
                                 gn_steps=40, pcg_per_step=2, traj_iters=1200, train_pcg=2)
-    print(json.dumps(line), flush=True)
+    emit(line)
 
 
 def main():
