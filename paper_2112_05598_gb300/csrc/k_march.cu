@@ -49,11 +49,9 @@ constexpr int kWarps = kThreads / 32;
 constexpr int kApplyCtas = 5;
 // the marches that read gather copies:
 constexpr int kApplyCopyCtas = 4;     // 5677; 5: 6222, 3: 6330
-// (A p from the store strides a resident grid over the tiles, and with 6 or 4
-// CTAs its stride met the rows of small images' costly tiles: 85^3, 64 x 53 x 100,
-// 3 A p: 1370 us with 5, 1820 with 6, 1630 with 4; 134^3, 59 x 141 x 272 9130,
-// 11660, 13950; 128^3, 4 x 800^2 11944, 11945, 12459.)
-constexpr int kStoreApplyCtas = 5;
+constexpr int kStoreApplyCtas = 6;    // 3 A p, 128^3, ms: 12 x 800^2 34.9; 5: 35.3; 20 x 400^2 14.4; 5: 16.2; 100 x 800^2 286; 5: 293
+                                      // (images below 3 pixels a voxel column, whose costly rows its stride
+                                      // met, do not come here: solver_copies in perf_api.cu)
 constexpr int kDiagCopyCtas = 4;      // 6628; 3: 6752, 2: 7964
 constexpr int kVjpCopyCtas = 4;       // vjp 97^3, 5 x 333 x 251: 1005; 3: 1091, 5: 1182
 constexpr int kJvpCopyCtas = 6;       // 6809; 5: 7018, 7: 7144, 4: 7729

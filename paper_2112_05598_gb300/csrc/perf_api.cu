@@ -476,9 +476,10 @@ int solver_spread(const perf_ctx* ctx) {
 
 // Whether they read copies: by the diagonal march, which runs in every step, and
 // where an image has 3 pixels a voxel column -- with fewer a warp's rays share
-// no lines, and A p from the store gains nothing from p's copy (us a step's 3 A p
-// without / with: 85^3, 53 x 100 1270 / 1370, 134^3, 141 x 272 8875 / 9130; 96^3,
-// 200^2 2530 / 2080, 64^3, 128^2 2640 / 2400, 128^3, 800^2 12290 / 11940).
+// no lines, and the stride of A p's resident grid can meet the images' costly
+// rows (us a step's 3 A p without / with: 85^3, 64 x 53 x 100 1270 / 1820, 134^3,
+// 59 x 141 x 272 8875 / 11660; 64^3, 32 x 128^2 2640 / 2300, 96^3, 12 x 200^2 2530 /
+// 2600 (its diagonal 1840 / 1270), 128^3, 4 x 800^2 12290 / 11940).
 bool solver_copies(const perf_ctx* ctx) {
     const perf::DevScene& d = ctx->ds;
     return solver_spread(ctx) && (double)d.W * d.H >= 3.0 * d.G * d.G && copies_pay(ctx, kDiag);
