@@ -27,7 +27,8 @@
  *           scene's dtype is PERF_BF16.
  * Pointers are DEVICE pointers unless a comment says HOST.  The caller owns
  * every buffer it passes in; the context owns only its workspace (PCG
- * vectors, residual buffer, FP64 scalars) and frees it in perf_destroy.
+ * vectors, residual buffer, FP64 scalars, gather copies of the grid) and frees
+ * it in perf_destroy.
  * Every call is asynchronous on the given stream (a cudaStream_t; NULL = the
  * legacy default stream) unless it writes a HOST output, in which case it
  * synchronises that stream before returning.

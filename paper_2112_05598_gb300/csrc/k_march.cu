@@ -1334,7 +1334,7 @@ static int grid_blocks(const void* fn, long long n_tiles, int cap_per_sm = 0) {
 // Up to kOneWarpTiles one tile a CTA, since four-warp CTAs leave the SMs with
 // one or two each (32^3, 8 x 64^2: the busiest SM had 1.9 times the mean work;
 // image 96^3, 16 x 64^2, 124 -> 113 us); above, the launches of the CTAs cost
-// more (image 128^3, 400^2: 122.4 against 120.7 us).  A CTA cap (tune_tiles)
+// more (image 128^3, 400^2: 122.4 against 120.7 us).  A CTA cap (perf_autotune)
 // needs the resident form, and a Gauss-Newton solve keeps it for its diagonal
 // (see launch_apply_coef_t).
 constexpr long long kOneWarpTiles = 152 * 20;
