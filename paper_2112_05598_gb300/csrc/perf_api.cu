@@ -460,6 +460,21 @@ int scatter_spread(const perf_ctx* ctx) {
     return perf::scatter_spread_of(ctx->ds.n_tiles, ctx->n_rays, ctx->n);
 }
 
+// Whether very many pixels of an image look through each voxel: tiles side by
+// side then add to the same few voxels, and on CTAs placed in order they do so
+// together.  A resident grid's drift apart (diagonal, us, in order / resident:
+// 28^3, 533 x 283 (192 pixels a voxel column) 7416 / 4449; 64^3, 800^2 (156) 4984
+// / 4054; 36^3, 354 x 208 (57) 4050 / 2937; below 32 in order by 2 to 12%; J^T v
+// and A p, whose reductions are fewer: in order by 3 to 13% up to 100, within 5%
+// either way above 128, where in order took up to 1.5 and 1.9 times the time
+// before it and resident at most 1.1).
+bool crowded(const perf_ctx* ctx, bool diag) {
+    const perf::DevScene& d = ctx->ds;
+    // (launches of one-warp CTAs, march_grid in k_march.cu, are too small for it)
+    return (d.n_tiles > 152 * 20 && (double)d.W * d.H >= (diag ? 50.0 : 100.0) * d.G * d.G) ||
+           (d.spread && !scatter_spread(ctx));
+}
+
 // scatter_spread for the marches of a solve: the diagonal and A p in the spread
 // order and from copies, or in the plain order from x and p on a resident grid,
 // which repeats its order of additions more closely from run to run (of the
@@ -486,25 +501,13 @@ bool solver_copies(const perf_ctx* ctx) {
 }
 
 // d for a solve's scatters without copies, resident where the spread order is
-// left for the plain one.
+// left for the plain one and in crowded scenes.
 void plain_scatter(const perf_ctx* ctx, perf::DevScene& d) {
     d.xcopy = nullptr;
     d.pcopy = nullptr;
     d.sigma8 = nullptr;
     d.spread = solver_spread(ctx);
-    if (ctx->ds.spread && !d.spread && d.cap_per_sm == 0) d.cap_per_sm = kResident;
-}
-
-// Whether very many pixels of an image look through each voxel: tiles side by
-// side then add to the same few voxels, and on CTAs placed in order they do so
-// together.  A resident grid's drift apart (diagonal, us, in order / resident:
-// 28^3, 533 x 283 (192 pixels a voxel column) 7416 / 4449; 64^3, 800^2 (156) 4984
-// / 4054; 36^3, 354 x 208 (57) 4050 / 2937; below 32 in order by 2 to 12%; J^T v
-// and A p, whose reductions are fewer, 5% either way above 128, and by 1.4 to 1.7
-// at worst in order).
-bool crowded(const perf_ctx* ctx) {
-    const perf::DevScene& d = ctx->ds;
-    return (double)d.W * d.H >= 100.0 * d.G * d.G || (d.spread && !scatter_spread(ctx));
+    if (d.cap_per_sm == 0 && (crowded(ctx, true) || (ctx->ds.spread && !d.spread))) d.cap_per_sm = kResident;
 }
 
 // d = the context's scene for march m with the gather copies of x (and of p, in
@@ -515,7 +518,7 @@ perf_status gather_copies(perf_ctx* ctx, const void* x, const void* p, int p_dty
     if (m != kForward && m != kJvp) {
         d.spread = scatter_spread(ctx);
         if (ctx->ds.spread && !d.spread) pay = false;
-        if (d.cap_per_sm == 0 && crowded(ctx)) d.cap_per_sm = kResident;
+        if (d.cap_per_sm == 0 && crowded(ctx, m == kDiag)) d.cap_per_sm = kResident;
     }
     const int parts = parts_of(m);
     if (!pay || !copies_room(ctx, parts, use)) return PERF_OK;
@@ -1073,7 +1076,7 @@ perf_status perf_gn_solve(perf_ctx* ctx, float* x, const void* target, int32_t n
             dl.xcopy = ctx->xcopy;
             dl.sigma8 = ctx->sigma8;
             dl.diag2 = ctx->diag2;
-            if (dl.cap_per_sm == 0 && crowded(ctx)) dl.cap_per_sm = kResident;
+            if (dl.cap_per_sm == 0 && crowded(ctx, true)) dl.cap_per_sm = kResident;
             // (its 4 CTAs an SM stride 2432 tiles, which in images that mostly miss
             // the grid met the costly rows again and again: 127^3, 16 x 79 x 648,
             // 2000 us with 4, 1100 with 3; elsewhere 4 are 2% faster)
